@@ -67,6 +67,16 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// The same, always accumulating, with the TMEM lanes whose bits are set in m0 .. m3
+// (lanes 0 .. 31, 32 .. 63, ..) left as they are.
+__device__ __forceinline__ void mma_bf16_lanes(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t m0,
+                                               uint32_t m1, uint32_t m2, uint32_t m3) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%4, %5, %6, %7}, p;\n\t}\n" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(idesc), "r"(m0), "r"(m1), "r"(m2), "r"(m3));
+}
+
 // The same with kind::f8f6f4 (8-bit operands, K = 32 per instruction).
 __device__ __forceinline__ void mma_f8(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
                                        uint32_t accumulate) {

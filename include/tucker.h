@@ -67,10 +67,14 @@ typedef enum {
 /* Element type of an input tensor.  Internal tensors are always float64. */
 typedef enum { TUCKER_F64 = 0, TUCKER_F32 = 1 } tucker_dtype;
 
-/* Arithmetic of the Gram and mode-product steps.  TUCKER_PREC_FP64 has
- * float64 accuracy: small products on the float64 pipe, large ones on the BF16
- * tensor cores with eight exact digits (56 bits) per entry, whose errors are no
- * larger.  TUCKER_PREC_BF16X4 ("BF16 digits") runs both on the BF16
+/* Arithmetic of the Gram and mode-product steps.  TUCKER_PREC_FP64:
+ * small products on the float64 pipe; large Grams, and large mode products with
+ * the factors, on the BF16 tensor cores with eight exact digits per entry: 56 bits
+ * below the largest magnitude of its row (Gram: over the columns of one work item)
+ * or of its column (product).  Their errors, relative to the norms of the two
+ * vectors multiplied, are no larger than those of chains of float64 multiply-adds;
+ * relative to sum |a_j b_j| they can be, where one vector's small entries meet the
+ * other's large ones.  TUCKER_PREC_BF16X4 ("BF16 digits") runs both on the BF16
  * tensor cores with exact integer digits: the Gram rounds every entry to 21
  * bits below the power of two above its row's largest magnitude in a group
  * of 512 columns and splits it into three balanced 7-bit digits (see
@@ -395,7 +399,9 @@ TUCKER_API int tucker_ttm_split(const void *Y, tucker_dtype dt, int64_t L, int64
  *   M is given column-major as either K x J (trans_m == 0, M[k,j] = Mp[k + K j]) or
  *   J x K and used transposed (trans_m != 0, M[k,j] = Mp[j + J k]; pass U_n with
  *   trans_m = 1 for the shrinking product Y x_n U_n^T).
- *   Y device (dt), M device float64, Z device float64 with L*K*B elements. */
+ *   Y device (dt), M device float64, Z device float64 with L*K*B elements.
+ *   M may select, permute or scale rows of any magnitude: every output has the
+ *   error of a chain of float64 multiply-adds, relative to sum_j |M[k, j] Y[j]|. */
 TUCKER_API int tucker_ttm(const void *Y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, const double *M, int64_t K,
                int trans_m, double *Z, void *stream);
 

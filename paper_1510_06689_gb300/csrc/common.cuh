@@ -165,8 +165,12 @@ int launch_gram_digits(const void *y, tucker_dtype dt, int64_t L, int64_t J, int
                        const DeviceInfo &dev, cudaStream_t s, Prof *prof, const int **redo, double **plain_ws);
 
 // Mode product Z(L,K,B) = sum_j A[k,j] Y(L,J,B) with A[k,j] = a[k*ak + j*aj].
+// normwise: an error of float64 rounding relative to |a_k| |y_c| will do, as it does
+// for products with orthonormal factors, whose own entries are that accurate.  Without
+// it the error is that of a chain of multiply-adds, relative to sum_j |a_kj y_jc|: a
+// caller's selection or scaling matrix keeps small entries whole beside large ones.
 int launch_ttm(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, const double *a, int64_t ak,
-               int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof);
+               int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof, bool normwise);
 // Same product, not stored: sum over all entries of (x - z)^2 into *d_out,
 // with x of the (L, K, B) shape.  d_partials holds ttm_diff_partials() doubles.
 int64_t ttm_diff_partials(int64_t L, int64_t J, int64_t B, int64_t K, const DeviceInfo &dev);
@@ -206,11 +210,14 @@ int launch_ttm_split(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64
                      const int *d_colexp = nullptr);
 // The float64 mode product from exact digits on the tensor cores: whether it
 // takes a size, the bytes of device scratch, and the launch; scratch[0] is then
-// the flag that tells the plain kernel to do the product after all.
-bool ttm_digits_applies(int64_t L, int64_t J, int64_t B, int64_t K);
+// the flag that tells the plain kernel to do the product after all.  Its error is
+// relative to the vectors' norms; without `normwise` the outputs for which that is
+// not enough are found and done again.
+bool ttm_digits_applies(int64_t L, int64_t J, int64_t B, int64_t K, bool normwise);
 int64_t ttm_digits_scratch(int64_t L, int64_t J, int64_t B, int64_t K, const DeviceInfo &dev);
 int launch_ttm_digits(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, const double *a, int64_t ak,
-                      int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, int *scratch);
+                      int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, int *scratch,
+                      bool normwise);
 // Eigensolver.  d_ws holds eig_workspace_doubles(J) doubles (0 when the
 // matrix fits in shared memory).  d_info holds 4 ints: [0] Jacobi sweeps,
 // [1] 0 if converged else 1, [2] the tucker_eig_path that ran, [3] the

@@ -470,7 +470,7 @@ int gram_typed(const T *y, int64_t L, int64_t J, int64_t B, double *d_S, double 
 
 template <typename T>
 int ttm_typed(const T *y, int64_t L, int64_t J, int64_t B, const double *a, int64_t ak, int64_t aj, int64_t K,
-              double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof) {
+              double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof, bool normwise) {
   TtmPlan p = ttm_plan<T, double, false>(L, J, B, K, dev);
   TK_CHECK(set_smem(k_ttm<T, double, false>, p.smem, dev));
   if (prof) prof->begin(TUCKER_PHASE_TTM);
@@ -482,12 +482,12 @@ int ttm_typed(const T *y, int64_t L, int64_t J, int64_t B, const double *a, int6
       if (p) cudaFreeAsync(p, s);
     }
   } scratch{nullptr, s};
-  if (ttm_digits_applies(L, J, B, K)) {
+  if (ttm_digits_applies(L, J, B, K, normwise)) {
     // on the tensor cores; the kernel below returns at once unless that one
     // could not take the values (an Inf or NaN, vectors near the underflow limit)
     TK_CUDA(cudaMallocAsync(&scratch.p, (size_t)ttm_digits_scratch(L, J, B, K, dev), s));
     TK_CHECK(launch_ttm_digits(y, sizeof(T) == 8 ? TUCKER_F64 : TUCKER_F32, L, J, B, a, ak, aj, K, z, dev, s,
-                               static_cast<int *>(scratch.p)));
+                               static_cast<int *>(scratch.p), normwise));
     only_if = static_cast<const int *>(scratch.p);
   }
   if (p.Kc > 0) {
@@ -621,10 +621,10 @@ int launch_gram(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B,
 }
 
 int launch_ttm(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, const double *a, int64_t ak,
-               int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof) {
+               int64_t aj, int64_t K, double *z, const DeviceInfo &dev, cudaStream_t s, Prof *prof, bool normwise) {
   if (dt == TUCKER_F64)
-    return ttm_typed(static_cast<const double *>(y), L, J, B, a, ak, aj, K, z, dev, s, prof);
-  return ttm_typed(static_cast<const float *>(y), L, J, B, a, ak, aj, K, z, dev, s, prof);
+    return ttm_typed(static_cast<const double *>(y), L, J, B, a, ak, aj, K, z, dev, s, prof, normwise);
+  return ttm_typed(static_cast<const float *>(y), L, J, B, a, ak, aj, K, z, dev, s, prof, normwise);
 }
 
 int64_t ttm_diff_partials(int64_t L, int64_t J, int64_t B, int64_t K, const DeviceInfo &dev) {

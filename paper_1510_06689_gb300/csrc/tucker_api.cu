@@ -715,7 +715,7 @@ static int sthosvd_impl(const void *X, tucker_dtype dt, const int64_t *dims, int
                                 &prof, want_colexp ? colexp.as<int>() : nullptr));
     else
       TK_CHECK(launch_ttm(Y, ydt, L, J, B, factor_bufs[n].as<double>(), /*ak=*/J, /*aj=*/1, R, ynew.as<double>(),
-                          dev, s, &prof));
+                          dev, s, &prof, true));
     // TUCKER_FAULT=timeout: raise the error flag a tensor-core wait raises on
     // expiry (host-side injection; no kernel is made to stall)
     if (fault_injection("timeout")) TK_CUDA(cudaMemsetAsync(d_terr, 1, 1, s));
@@ -800,7 +800,7 @@ static int expand_modes(const tucker_result *r, int skip, double *final_out, Dev
     }
     // A = rows lo[n].. of U_n (I_n x J, column-major): A[k, j] = U[lo + k + I_n j]
     TK_CHECK(launch_ttm(y, TUCKER_F64, L, J, B, r->factors[n] + (lo ? lo[n] : 0), /*ak=*/1, /*aj=*/r->dims[n], K, z,
-                        dev, s, prof));
+                        dev, s, prof, true));
     if (!(final_out && k == cnt - 1)) {
       tmp.reset();
       tmp.p = next.release();
@@ -884,7 +884,7 @@ static int hooi_iterate(const void *X, tucker_dtype dt, int max_iters, double to
         TK_CHECK(launch_ttm_split(Y, ydt, L, J, B, out->factors[m], R, ynew.as<double>(), d_terr, dev, s, &prof));
       else
         TK_CHECK(launch_ttm(Y, ydt, L, J, B, out->factors[m], /*ak=*/J, /*aj=*/1, R, ynew.as<double>(), dev, s,
-                            &prof));
+                            &prof, true));
       ybuf.reset();
       ybuf.p = ynew.release();
       ybuf.s = s;
@@ -948,7 +948,7 @@ static int hooi_iterate(const void *X, tucker_dtype dt, int max_iters, double to
       }
       TK_CUDA(cudaMemcpyAsync(out->factors[n], V.p, sizeof(double) * J * R, cudaMemcpyDeviceToDevice, s));
       if (n == N - 1) {  // G = Y x_{N-1} U_{N-1}^T
-        TK_CHECK(launch_ttm(Y, ydt, L, J, B, out->factors[n], /*ak=*/J, /*aj=*/1, R, out->core, dev, s, &prof));
+        TK_CHECK(launch_ttm(Y, ydt, L, J, B, out->factors[n], /*ak=*/J, /*aj=*/1, R, out->core, dev, s, &prof, true));
       }
     }
     double f = 0.0;
@@ -1835,7 +1835,7 @@ int tucker_ttm(const void *Y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, 
   TK_CHECK(device_info(&dev));
   Prof prof(s);
   const int64_t ak = trans_m ? J : 1, aj = trans_m ? 1 : K;
-  TK_CHECK(launch_ttm(Y, dt, L, J, B, M, ak, aj, K, Z, dev, s, &prof));
+  TK_CHECK(launch_ttm(Y, dt, L, J, B, M, ak, aj, K, Z, dev, s, &prof, false));
   if (prof.on) {
     TK_CUDA(cudaStreamSynchronize(s));
     prof.flush();

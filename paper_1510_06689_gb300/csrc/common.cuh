@@ -93,6 +93,11 @@ void batched_last_tuning(int64_t *kc, int *grid, float *ms6);
 // ---------------------------------------------------------------------------
 // device description (cached per device)
 // ---------------------------------------------------------------------------
+// Stream-ordered device memory for a faster way of what also works without it:
+// *p = nullptr (and TUCKER_OK) when the device has none left, or when `s` is being
+// captured (a graph then holds kernels only).
+int optional_scratch(void **p, size_t bytes, cudaStream_t s);
+
 struct DeviceInfo {
   int device = -1;
   int sms = 0;
@@ -152,9 +157,10 @@ int launch_norm2(const void *x, tucker_dtype dt, int64_t n, double *d_partials, 
 
 // Gram of the (L, J, B) view into d_S (J x J, both triangles).  d_ws holds
 // gram_workspace_doubles() doubles of split-K partials.
-int64_t gram_workspace_doubles(int64_t L, int64_t J, int64_t B, const DeviceInfo &dev);
+// digits: on the tensor cores (where gram_digits_applies), which takes more workspace.
+int64_t gram_workspace_doubles(int64_t L, int64_t J, int64_t B, const DeviceInfo &dev, bool digits);
 int launch_gram(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, double *d_S, double *d_ws,
-                const DeviceInfo &dev, cudaStream_t s, Prof *prof);
+                const DeviceInfo &dev, cudaStream_t s, Prof *prof, bool digits);
 // The float64 Gram from exact digits on the tensor cores: whether it takes a
 // size, its workspace (given the plain kernel's), and the launch, which leaves
 // in *redo the device flag that tells the plain kernel (workspace *plain_ws) to

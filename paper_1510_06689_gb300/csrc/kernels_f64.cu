@@ -434,10 +434,10 @@ int set_smem(K kernel, size_t bytes, const DeviceInfo &dev) {
 
 template <typename T>
 int gram_typed(const T *y, int64_t L, int64_t J, int64_t B, double *d_S, double *d_ws, const DeviceInfo &dev,
-               cudaStream_t s, Prof *prof) {
+               cudaStream_t s, Prof *prof, bool digits) {
   GramPlan p = gram_plan(L, J, B, dev);
   TK_CHECK(set_smem(k_gram_partial<T>, p.smem, dev));
-  if (gram_digits_applies(L, J, B)) {
+  if (digits) {
     // on the tensor cores; the kernels below return at once unless that one
     // could not take the values (an Inf or NaN, rows near the underflow limit)
     const int *redo = nullptr;
@@ -482,10 +482,11 @@ int ttm_typed(const T *y, int64_t L, int64_t J, int64_t B, const double *a, int6
       if (p) cudaFreeAsync(p, s);
     }
   } scratch{nullptr, s};
-  if (ttm_digits_applies(L, J, B, K, normwise)) {
+  if (ttm_digits_applies(L, J, B, K, normwise))
+    TK_CHECK(optional_scratch(&scratch.p, (size_t)ttm_digits_scratch(L, J, B, K, dev), s));
+  if (scratch.p) {
     // on the tensor cores; the kernel below returns at once unless that one
     // could not take the values (an Inf or NaN, vectors near the underflow limit)
-    TK_CUDA(cudaMallocAsync(&scratch.p, (size_t)ttm_digits_scratch(L, J, B, K, dev), s));
     TK_CHECK(launch_ttm_digits(y, sizeof(T) == 8 ? TUCKER_F64 : TUCKER_F32, L, J, B, a, ak, aj, K, z, dev, s,
                                static_cast<int *>(scratch.p), normwise));
     only_if = static_cast<const int *>(scratch.p);
@@ -608,16 +609,16 @@ int fp64_peak(double *tflops, double *ms_out, const DeviceInfo &dev, cudaStream_
   return TUCKER_OK;
 }
 
-int64_t gram_workspace_doubles(int64_t L, int64_t J, int64_t B, const DeviceInfo &dev) {
+int64_t gram_workspace_doubles(int64_t L, int64_t J, int64_t B, const DeviceInfo &dev, bool digits) {
   GramPlan p = gram_plan(L, J, B, dev);
   const int64_t plain = (int64_t)std::max(p.nsplit, 1) * p.n_micro * 16;
-  return gram_digits_applies(L, J, B) ? gram_digits_workspace(L, J, B, dev, plain) : plain;
+  return digits ? gram_digits_workspace(L, J, B, dev, plain) : plain;
 }
 
 int launch_gram(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, double *d_S, double *d_ws,
-                const DeviceInfo &dev, cudaStream_t s, Prof *prof) {
-  if (dt == TUCKER_F64) return gram_typed(static_cast<const double *>(y), L, J, B, d_S, d_ws, dev, s, prof);
-  return gram_typed(static_cast<const float *>(y), L, J, B, d_S, d_ws, dev, s, prof);
+                const DeviceInfo &dev, cudaStream_t s, Prof *prof, bool digits) {
+  if (dt == TUCKER_F64) return gram_typed(static_cast<const double *>(y), L, J, B, d_S, d_ws, dev, s, prof, digits);
+  return gram_typed(static_cast<const float *>(y), L, J, B, d_S, d_ws, dev, s, prof, digits);
 }
 
 int launch_ttm(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, const double *a, int64_t ak,

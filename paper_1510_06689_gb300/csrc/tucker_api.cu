@@ -245,6 +245,36 @@ static int fault_injection(const char *what) {
   return f && strcmp(f, what) == 0;
 }
 
+int optional_scratch(void **p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  TK_CUDA(cudaStreamIsCapturing(s, &capturing));
+  if (capturing != cudaStreamCaptureStatusNone || fault_injection("scratch")) return TUCKER_OK;
+  const cudaError_t e = cudaMallocAsync(p, bytes, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    *p = nullptr;
+    return TUCKER_OK;
+  }
+  TK_CUDA(e);
+  return TUCKER_OK;
+}
+
+// The float64 Gram with its workspace in `ws`: on the tensor cores where that applies
+// and there is memory for its exponent table and partial sums.
+static int gram_f64(const void *y, tucker_dtype dt, int64_t L, int64_t J, int64_t B, double *S, DevBuf &ws,
+                    const DeviceInfo &dev, cudaStream_t s, Prof *prof) {
+  ws.reset();
+  bool digits = gram_digits_applies(L, J, B);
+  if (digits) {
+    ws.s = s;
+    TK_CHECK(optional_scratch(&ws.p, sizeof(double) * gram_workspace_doubles(L, J, B, dev, true), s));
+    digits = ws.p != nullptr;
+  }
+  if (!digits) TK_CHECK(ws.alloc(sizeof(double) * gram_workspace_doubles(L, J, B, dev, false), s));
+  return launch_gram(y, dt, L, J, B, S, ws.as<double>(), dev, s, prof, digits);
+}
+
 // ---------------------------------------------------------------------------
 // argument checks
 // ---------------------------------------------------------------------------
@@ -652,9 +682,7 @@ static int sthosvd_impl(const void *X, tucker_dtype dt, const int64_t *dims, int
         TK_CHECK(set_norm(h[0]));
       }
     } else {
-      const int64_t gws = gram_workspace_doubles(L, J, B, dev);
-      TK_CHECK(gramws.alloc(sizeof(double) * gws, s));
-      TK_CHECK(launch_gram(Y, ydt, L, J, B, S.as<double>(), gramws.as<double>(), dev, s, &prof));
+      TK_CHECK(gram_f64(Y, ydt, L, J, B, S.as<double>(), gramws, dev, s, &prof));
     }
     // eigenvector step
     const int64_t ews = eig_workspace_doubles(J);
@@ -933,8 +961,7 @@ static int hooi_iterate(const void *X, tucker_dtype dt, int max_iters, double to
       for (int q = 0; q < n; ++q) L *= cur[q];
       for (int q = n + 1; q < N; ++q) B *= cur[q];
       const int64_t J = out->dims[n], R = out->ranks[n];
-      TK_CHECK(gramws.alloc(sizeof(double) * gram_workspace_doubles(L, J, B, dev), s));
-      TK_CHECK(launch_gram(Y, ydt, L, J, B, S.as<double>(), gramws.as<double>(), dev, s, &prof));
+      TK_CHECK(gram_f64(Y, ydt, L, J, B, S.as<double>(), gramws, dev, s, &prof));
       const int64_t ews = eig_workspace_doubles(J);
       if (ews > 0) TK_CHECK(eigws.alloc(sizeof(double) * ews, s));
       TK_CHECK(launch_eig(S.as<double>(), J, lam.as<double>(), V.as<double>(), ews > 0 ? eigws.as<double>() : nullptr,
@@ -1694,8 +1721,7 @@ int tucker_gram(const void *Y, tucker_dtype dt, int64_t L, int64_t J, int64_t B,
   TK_CHECK(device_info(&dev));
   Prof prof(s);
   DevBuf ws;
-  TK_CHECK(ws.alloc(sizeof(double) * gram_workspace_doubles(L, J, B, dev), s));
-  TK_CHECK(launch_gram(Y, dt, L, J, B, S, ws.as<double>(), dev, s, &prof));
+  TK_CHECK(gram_f64(Y, dt, L, J, B, S, ws, dev, s, &prof));
   if (prof.on) {
     TK_CUDA(cudaStreamSynchronize(s));
     prof.flush();

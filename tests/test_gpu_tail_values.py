@@ -29,3 +29,13 @@ def test_tail_sum(gpu_lib, J, wide):
     lam, got = _tail(gpu_lib, J, wide)
     print(f"J={J} wide={wide}: sum off by {abs(got[8:].sum() - lam[8:].sum()) / (J * U * lam[0]):.2f} J u lambda_1")
     assert abs(got[8:].sum() - lam[8:].sum()) <= 4 * J * U * lam[0]
+
+
+@pytest.mark.parametrize("wide", [1e-4, 1e-5, 1e-6, 1e-7, 1e-9])
+@pytest.mark.parametrize("J", [64, 100, 200, 400])
+def test_tail_values_one_by_one(gpu_lib, J, wide):
+    """Every value within J u lambda_1 of its own, the rounding of a float64 solve (and as much for the tensor's), whether
+    float32 stage, Rayleigh quotients or a level of its own gave it."""
+    lam, got = _tail(gpu_lib, J, wide)
+    print(f"J={J} wide={wide}: values off by {np.abs(got - lam).max() / (J * U * lam[0]):.2f} J u lambda_1")
+    assert np.abs(got - lam).max() <= 2 * J * U * lam[0]

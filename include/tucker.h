@@ -121,14 +121,16 @@ typedef struct tucker_result {
                                          unresolved (Algorithm 1 needs only the leading R_n
                                          eigenvectors and the discarded sum): its entries are
                                          then Rayleigh quotients of a basis of its invariant
-                                         subspace, and every sum from the cut on stays exact */
+                                         subspace, or (tucker_sthosvd_batched) eigenvalues to
+                                         ~2^-20 of the largest of them, and every sum from the
+                                         cut on stays exact */
   double tail[TUCKER_MAX_MODES];      /* discarded eigenvalue sum per mode (clamped at 0) */
   double norm2_x;                     /* ||X||^2 */
   double threshold;                   /* eps^2 ||X||^2 / N (0 when eps <= 0) */
   int eig_path[TUCKER_MAX_MODES];     /* tucker_eig_path of each mode's eigensolve */
   int eig_resolved[TUCKER_MAX_MODES]; /* leading eigenvalues of mode n resolved one by one (I_n unless a
-                                         tail cluster was left unresolved; eigvals past this count are
-                                         Rayleigh quotients whose sum is exact) */
+                                         tail cluster was left unresolved; of eigvals past this count
+                                         the sum is exact, see there) */
   void *priv;                         /* library bookkeeping; do not touch */
 } tucker_result;
 

@@ -279,6 +279,11 @@ int launch_jacobi32_batched(const double *const *d_A, const int *d_J, double *co
 // order, for the eigenvalues above what float32 resolves.
 int launch_eig32_lead_batched(const double *const *d_A, const int *d_J, double *const *d_X, int *d_nlead, int count,
                               int maxJ, cudaStream_t s);
+// The float32 stage's eigenvalues of `count` tails (J <= 128): with m = d_info[4 b + 2]
+// >= 2, lam_b[J_b - m ..] = the m largest of A_b (ld J_b), moved to the sum of what is
+// there (m times their mean).
+int launch_eig32_tail_batched(const double *const *d_A, const int *d_J, const int *d_info, double *const *d_lam,
+                              int count, int maxJ, cudaStream_t s);
 // Rank rule: *d_rank = R, *d_tail = discarded sum.
 int launch_rank_cut(const double *d_lam, int64_t J, double threshold, int keep_all, int64_t *d_rank,
                     double *d_tail, cudaStream_t s, Prof *prof);

@@ -41,3 +41,28 @@ def test_batched_mixed_range(gpu_lib, dims):
     m = x.reshape(dims[0], -1, order="F")
     lam = np.linalg.eigvalsh(m @ m.T)[::-1]
     assert np.abs(np.array(res.eigvals[0]) - lam).max() <= 4 * dims[0] * 2.0 ** -53 * lam[0]
+
+
+@pytest.mark.parametrize("count", [1, 40])
+def test_batched_tail_values(gpu_lib, count):
+    """Past the rank cut each eigenvalue is its own: within 2^-18 of the tail's largest (float32's 2^-22, a few times)
+    and the solves' 1e-12 lambda_1 of the oracle's, in order."""
+    import oracle
+    from synthetic import tucker_tensor_np
+
+    shapes = [((128, 40, 9), (5, 4, 3)), ((33, 64, 65), (16, 8, 8)), ((31, 17, 100), (8, 8, 8)), ((24, 3, 70), (4, 2, 6)),
+              ((70, 60, 50), (30, 30, 30))]
+    xs, dims = [], []
+    for i in range(count):
+        d, r = shapes[i % len(shapes)]
+        xs.append(tucker_tensor_np(d, r, seed=3, tensor=i, noise=3e-4, decay=0.15 * (max(r) == 30)))
+        dims.append(d)
+    res = gpu_lib.sthosvd_batched([torch.from_numpy(x).cuda() for x in xs], dims, 1e-2)
+    for i in range(min(count, len(shapes))):
+        ref = oracle.sthosvd(xs[i], dims[i], 1e-2)
+        assert res[i].ranks == ref["ranks"]
+        for n, J in enumerate(dims[i]):
+            lam, got, k = np.array(ref["eigvals"][n]), np.array(res[i].eigvals[n]), res[i].ranks[n]
+            if k < J:
+                assert np.abs(got - lam).max() <= 2.0 ** -18 * lam[k] + 1e-12 * lam[0]
+                assert (np.diff(got) <= 1e-12 * lam[0]).all()

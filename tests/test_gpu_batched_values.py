@@ -66,3 +66,20 @@ def test_batched_tail_values(gpu_lib, count):
             if k < J:
                 assert np.abs(got - lam).max() <= 2.0 ** -18 * lam[k] + 1e-12 * lam[0]
                 assert (np.diff(got) <= 1e-12 * lam[0]).all()
+
+
+@pytest.mark.parametrize("dims", [(20, 18, 16), (70, 40, 30)])
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_batched_non_finite_tensor(gpu_lib, bad, dims):
+    """The call succeeds; the tensor's own norm is not finite, and the others come out as without it, bit for bit."""
+    rng = np.random.default_rng(2)
+    xs = [rng.standard_normal(int(np.prod(dims))) for _ in range(3)]
+    ok = gpu_lib.sthosvd_batched([torch.from_numpy(x).cuda() for x in xs], [dims] * 3, 1e-3)
+    xs[1][777] = bad
+    res = gpu_lib.sthosvd_batched([torch.from_numpy(x).cuda() for x in xs], [dims] * 3, 1e-3)
+    assert not np.isfinite(res[1].norm2)
+    for i in (0, 2):
+        assert res[i].ranks == ok[i].ranks and torch.equal(res[i].core(), ok[i].core())
+        for n in range(3):
+            assert torch.equal(res[i].factor(n), ok[i].factor(n))
+            assert np.array_equal(res[i].eigvals[n], ok[i].eigvals[n])

@@ -12,6 +12,9 @@ so no flush is needed between steps.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
 
+prints one JSON line with the headline figures; the whole record (phases,
+rooflines, the other workloads) goes to stderr as one more.
+
 N > 1 runs N independent replicas (one per GPU, launched by torchrun); the
 single-tensor method has an all-reduce in every Gram, so it is not sharded.
 --impl reference times the CPU oracle on the host cores on a bounded sample
@@ -295,6 +298,24 @@ def config_dict(w, eps, precision):
         "input_bytes": w.nbytes, "l2_policy": f"input {w.nbytes / 1e9:.1f} GB >> 129 MB L2 (no flush needed)",
         "parallelism": "replicas (one independent tensor per GPU)",
     }
+
+
+def headline(line):
+    """The measurements that the bench is run for, short enough for a log that keeps little of the output; the whole
+    record, with the tables of the other workloads, goes to stderr before it."""
+    keep = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gram_tflops", "ranks", "rel_error", "equal_rel_error",
+            "gpu_launches", "clocks")
+    out = {k: line[k] for k in keep if k in line}
+    part = {"methods": ("value", "ms_per_step"),
+            "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step", "precision"),
+            "cpu_baseline": ("value", "unit", "cores", "kind")}
+    for k, names in part.items():
+        if k in line:
+            rows = line[k].items() if k == "methods" else [(None, line[k])]
+            rows = {m: {n: r[n] for n in names if n in r} for m, r in rows}
+            out[k] = rows if k == "methods" else rows[None]
+    return out
 
 
 def time_method(tucker, x, dims, eps, precision, steps, warmup, world, local, stream):
@@ -928,7 +949,8 @@ def main():
         except Exception as e:  # recorded in the line; the headline measurement above stands
             line["next_rows"]["paper_shapes"] = {"error": f"{type(e).__name__}: {e}"}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)  # every table
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         import torch.distributed as dist
 

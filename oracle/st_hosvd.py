@@ -126,7 +126,8 @@ def leading_eigenpairs(s):
     v = v[:, order]
     for c in range(v.shape[1]):
         col = v[:, c]
-        r = int(np.argmax(np.abs(col)))  # first (lowest) row on ties
+        mag = np.abs(col)
+        r = int(np.argmax(mag >= mag.max() * (1 - 1e-14)))  # first (lowest) row on ties, up to LAPACK's rounding
         if col[r] < 0:
             v[:, c] = -col
     return lam, v

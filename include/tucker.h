@@ -305,8 +305,8 @@ TUCKER_API int tucker_rel_error(const void *X, tucker_dtype dt, const tucker_res
 /*
  * tucker_result_copy -- the core (mode -1, natural layout) or factor U_mode (0-based,
  * row-major I_mode x R_mode: out[i R_mode + r]) of a device-resident result into the
- * caller's device buffer, one kernel on `stream` of the result's device (the current
- * one).  Returns TUCKER_OK, EINVAL, ECUDA, or EUNSUPPORTED when the result lives on
+ * caller's device buffer, one copy (core) or kernel (factor) on `stream` of the result's
+ * device (the current one).  Returns TUCKER_OK, EINVAL, ECUDA, or EUNSUPPORTED when the result lives on
  * another device or on the host.  Stream-ordered; does not synchronise.
  */
 TUCKER_API int tucker_result_copy(const tucker_result *r, int mode, double *out, void *stream);
@@ -412,7 +412,9 @@ TUCKER_API int tucker_ttm(const void *Y, tucker_dtype dt, int64_t L, int64_t J, 
  * callers such as a process whose framework has already reserved nearly all
  * of the GPU's memory for its own pool, or code that must not trigger the
  * device-wide synchronisation that cudaMalloc/cudaFree can cause.
- *   Same arguments, layout and result as tucker_gram (the caller passes Y and S).
+ *   Same arguments, layout and output as tucker_gram (the caller passes Y and S),
+ *   by the plain float64 kernels at every size: where tucker_gram takes the digits
+ *   on the tensor cores, the two differ by their rounding.
  *   The split-K partial sums live in a static device array of
  *   TUCKER_NOALLOC_SCRATCH_BYTES that each GPU loading the library holds until
  *   the process exits; the call allocates nothing.  Requests whose partial sums
@@ -457,9 +459,9 @@ TUCKER_API int tucker_memory_stats(int64_t *pool_used, int64_t *pool_reserved, i
 TUCKER_API int tucker_memory_trim(void);
 
 /* The tuning of the last batched device pipeline: columns per work item, the
- * mode product's persistent CTAs, and six times in ms (512 / 2048 / 8192
- * columns, each twice: the first mode's Gram).  Any pointer may be
- * NULL.  Host only. */
+ * mode product's persistent CTAs, and the first mode's Gram in ms with 512, 2048 and
+ * 8192 columns per item, each in two neighbouring places of the six (the second is a
+ * copy of the first).  Any pointer may be NULL.  Host only. */
 TUCKER_API void tucker_batched_tuning(int64_t *cols_per_item, int *ctas, float *candidate_ms);
 
 /* Float64 throughput of the current GPU: a register-resident loop of

@@ -251,7 +251,7 @@ struct EigTail {
 int launch_eig(const double *d_S, int64_t J, double *d_lam, double *d_V, double *d_ws, int *d_info,
                cudaStream_t s, Prof *prof, double tail_budget = -1.0, int need = 0, EigTail *tail = nullptr);
 // Mixed-precision eigensolver (float32 first stage + float64 refinement,
-// J <= 128): *verified = 1 when lam, V and d_info hold a result that passed the
+// J <= 512): *verified = 1 when lam, V and d_info hold a result that passed the
 // device check; otherwise the caller runs the float64 Jacobi.  Synchronises s.
 int launch_eig_mp(const double *d_S, int64_t J, double *d_lam, double *d_V, int *d_info, int *verified,
                   cudaStream_t s, Prof *prof, double tail_budget = -1.0, int need = 0, EigTail *tail = nullptr);

@@ -419,7 +419,6 @@ static void free_result_device(tucker_result *r, cudaStream_t *own = nullptr) {
 }
 
 namespace {
-// trace of a J x J column-major matrix, summed in index order (one thread)
 // out (row-major I x R) = U (column-major), by 32 x 32 tiles through shared memory.
 __global__ void __launch_bounds__(256) k_transpose(const double *__restrict__ U, int I, int R,
                                                    double *__restrict__ out) {
@@ -432,6 +431,7 @@ __global__ void __launch_bounds__(256) k_transpose(const double *__restrict__ U,
     if (i0 + k < I && r0 + tx < R) out[(int64_t)(i0 + k) * R + r0 + tx] = t[tx][k];
 }
 
+// trace of a J x J column-major matrix, summed in index order (one thread)
 __global__ void k_trace(const double *__restrict__ S, int J, double *__restrict__ out) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double t = 0.0;

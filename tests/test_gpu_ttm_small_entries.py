@@ -58,3 +58,18 @@ def test_products_with_factors(gpu_lib, dims, ranks, dt):
     y = gpu_lib.reconstruct(res).cpu().numpy().reshape(dims, order="F")
     bound = 1.3 * U * float(np.linalg.norm(got)) * sum(np.sqrt(d) * r for d, r in zip(dims, ranks))
     assert float(np.sqrt(((y - back) ** 2).sum())) <= bound
+
+
+@pytest.mark.parametrize("C", [32, 127, 300])
+@pytest.mark.parametrize("J,K", [(64, 33), (128, 128), (300, 200), (512, 512)])
+def test_ttm_few_columns(gpu_lib, J, K, C):
+    """Few columns, the rows of the small sums spread over CTAs: dense, graded and sparse rows of one matrix, each output
+    within the chain's bound of test_ttm_small_entries."""
+    rng = np.random.default_rng([J, K, C])
+    y = rng.standard_normal((C, J)) * 10.0 ** rng.uniform(-12, 4, J)
+    m = rng.standard_normal((K, J))
+    m[1::3] *= 10.0 ** rng.uniform(-8, 8, J)
+    m[2::3] *= rng.random((len(m[2::3]), J)) < 0.1
+    z = gpu_lib.ttm(torch.from_numpy(y.reshape(-1).copy()).cuda(), 1, J, C, torch.from_numpy(m).cuda()).cpu().numpy()
+    ref, mag = y @ m.T, np.abs(y) @ np.abs(m).T
+    assert (np.abs(z.reshape(C, K) - ref) <= 2 * (J + 1) * U * mag).all()
